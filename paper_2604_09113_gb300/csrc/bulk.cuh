@@ -46,6 +46,14 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
   }
 }
 
+// mbar_wait by all 32 lanes of a warp, with one answer for all of them: a lane
+// that left a loop alone would leave the others waiting for it in the next
+// full-mask operation, which no limit ends.  The vote also brings the lanes
+// together, as the .sync.aligned tensor-memory instructions behind it ask.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, volatile int* abort_flag = nullptr) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag));
+}
+
 // dst (shared, 16-byte aligned) <- bytes at src (global, 16-byte aligned);
 // bytes a multiple of 16.
 __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {

@@ -312,10 +312,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1) assemble_tc_kernel(TcParams P) 
     const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
     const long long kp = (long long)P.ndof * (P.ndof + 1) / 2;
     double* Kc = P.Kout + cell * kp;
-    for (int t = 0; t < T && !s_abort; ++t) {
+    // every way out of these loops is taken by whole warps (mbar_wait_warp)
+    for (int t = 0; t < T; ++t) {
       const int b = t & 1;
-      if (!mbar_wait(&bar_accfull[b], (uint32_t)((t >> 1) & 1), &s_abort) ||
-          !mbar_wait(&bar_u1full[b], (uint32_t)((t >> 1) & 1), &s_abort)) {
+      if (!mbar_wait_warp(&bar_accfull[b], (uint32_t)((t >> 1) & 1), &s_abort) ||
+          !mbar_wait_warp(&bar_u1full[b], (uint32_t)((t >> 1) & 1), &s_abort)) {
         s_abort = 1;
         atomicOr(P.err, 8);
         break;
@@ -352,28 +353,30 @@ __global__ void __launch_bounds__(TC_THREADS, 1) assemble_tc_kernel(TcParams P) 
         mine[row] = g ? make_float2(vh[0], vl[0]) : make_float2(vh[2], vl[2]);
         mine[TC_M + row] = g ? make_float2(vh[1], vl[1]) : make_float2(vh[3], vl[3]);
         mbar_arrive(&bar_xch[par]);
-        if (!mbar_wait(&bar_xch[par], (uint32_t)((pr >> 1) & 1), &s_abort)) {
+        if (!mbar_wait_warp(&bar_xch[par], (uint32_t)((pr >> 1) & 1), &s_abort)) {
           s_abort = 1;
           atomicOr(P.err, 16);
           ok = false;
           break;
         }
-        if (!act) continue;
-        const float2* other = xch + (size_t)(2 * par + (1 - g)) * 2 * TC_M;
-        const int2 kk = P.pairs[pr];
-        const long long r = 2 * kk.x + g, q0 = 2 * kk.y;
-        double* Kr = Kc + r * P.ndof - r * (r - 1) / 2 - r;
-        // (h, l) + (w.x, w.y) in double-float (two-sum of the high words)
-        auto combine = [](float h, float l, float2 w) {
-          const float sh = __fadd_rn(h, w.x), bb = __fsub_rn(sh, h);
-          const float er = __fadd_rn(__fsub_rn(h, __fsub_rn(sh, bb)), __fsub_rn(w.x, bb));
-          const float sl = __fadd_rn(__fadd_rn(l, w.y), er);
-          return (double)sh + (double)sl;
-        };
-        const double out0 = combine(kh0, kl0, other[row]);
-        const double out1 = combine(kh1, kl1, other[TC_M + row]);
-        if (!(kk.x == kk.y && g == 1)) Kr[q0] = out0;
-        Kr[q0 + 1] = out1;
+        if (act) {
+          const float2* other = xch + (size_t)(2 * par + (1 - g)) * 2 * TC_M;
+          const int2 kk = P.pairs[pr];
+          const long long r = 2 * kk.x + g, q0 = 2 * kk.y;
+          double* Kr = Kc + r * P.ndof - r * (r - 1) / 2 - r;
+          // (h, l) + (w.x, w.y) in double-float (two-sum of the high words)
+          auto combine = [](float h, float l, float2 w) {
+            const float sh = __fadd_rn(h, w.x), bb = __fsub_rn(sh, h);
+            const float er = __fadd_rn(__fsub_rn(h, __fsub_rn(sh, bb)), __fsub_rn(w.x, bb));
+            const float sl = __fadd_rn(__fadd_rn(l, w.y), er);
+            return (double)sh + (double)sl;
+          };
+          const double out0 = combine(kh0, kl0, other[row]);
+          const double out1 = combine(kh1, kl1, other[TC_M + row]);
+          if (!(kk.x == kk.y && g == 1)) Kr[q0] = out0;
+          Kr[q0 + 1] = out1;
+        }
+        __syncwarp();
       }
       if (!ok) break;
       tc_fence_before();

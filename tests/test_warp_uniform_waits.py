@@ -23,7 +23,7 @@ def _epilogue(name):
     return src[start:i]
 
 
-@pytest.mark.parametrize("name", ["assemble_digits.cu"])
+@pytest.mark.parametrize("name", ["assemble_digits.cu", "assemble_tc.cu"])
 def test_epilogue_leaves_as_a_warp(name):
     body = _epilogue(name)
     assert not re.search(r"\bmbar_wait\(", body), "a lane's own wait: use mbar_wait_warp"

@@ -190,8 +190,8 @@ struct romb_ctx {
   // per-cell arrays
   double* d_chat = nullptr;     // [cells][nL][16]
   float* d_chat32 = nullptr;    // [cells][144] FP32 copy for the tensor-core epilogue
-  double* d_gq = nullptr;       // [cells][9][2][2][hi, lo] sqrt(det J) J^-1 (in the memory of d_G)
-  uint32_t* d_cdig = nullptr;   // [cells][528] digits of theta and G' of the FP64 form (in the memory of d_S)
+  double* d_gq = nullptr;       // [cells][9][2][2][hi, lo] sqrt(det J) J^-1 (in the memory of d_W)
+  uint32_t* d_cdig = nullptr;   // [cells][528] digits of theta and G' of the FP64 form (in the memory of d_Phi)
   double* d_theta = nullptr;    // [cells][kmax]
   int2* d_wts = nullptr;        // [cells][4][12] 1D interpolation weights, fixed point (in the memory of d_W)
   unsigned char* d_fams = nullptr;    // model table of launch_theta

@@ -134,7 +134,7 @@ romb_status romb_train_load(romb_ctx* ctx, const char* rom_path, int* family_out
  * theta = ((1-rho) I_r(mu), rho) from the MDEIM interpolation of the cell's
  * family, Chat at the (q+1)^2 interpolation nodes (Eq. FAST interpolation), and
  * the contraction K = sum_{j1 j2 k3} [U_r I_r (1-rho) + rho I_Pi] C.
- * Every form interpolates theta in 56-bit fixed point (within the rounding of
+ * Every form interpolates theta in 59-bit fixed point (within the rounding of
  * the FP64 sums).  prec = ROMB_FP64: the contraction by exact products of 8-bit
  * digits on the tensor cores, to the rounding of FP64 sums, or by FP64 FMAs
  * where the digits' memory cannot be had (romb_set_fp64_arithmetic asks for
@@ -253,7 +253,7 @@ enum { ROMB_PRECOND_AUTO = -1, ROMB_PRECOND_FP64 = 0, ROMB_PRECOND_FP32 = 1 };
 romb_status romb_set_precond_precision(romb_ctx* ctx, int mode);
 
 /* The arithmetic of the FP64 form from the next romb_assemble on.  0 (default):
- * theta in 56-bit fixed point, the contraction by exact digit products on the
+ * theta in 59-bit fixed point, the contraction by exact digit products on the
  * tensor cores, and the matrix products of romb_factor in 56-bit integers, each
  * within the rounding of the FP64 sums.  1: all on the FP64 pipe, every sum in
  * one fixed order (the assembly at ~10 times the time).  The two

@@ -19,7 +19,7 @@
 
 struct RomDev {
   const int2* At;        // [ngrid][n_r] interpolation samples, fixed point (fx56.cuh): A_t 2^-at_exp[t]
-  const int* at_exp;     // [n_r] exponents with |A_t| <= 2^(at_exp - 2)
+  const int* at_exp;     // [n_r] exponents with |A_t| <= 2^(at_exp - 1)
   int n_r, r;
   double lo4[4], hi4[4]; // the cluster's box per threshold
   double g01[12];        // degree-r GLL nodes of [0, 1]; node i of threshold d is lo4 + (hi4 - lo4) g01[i]
@@ -186,7 +186,7 @@ __global__ void __launch_bounds__(128) cell_prep_kernel(CellParams P, const Thet
     for (int i = 0; i < n1; ++i) nodes[i] = R.lo4[d] + (R.hi4[d] - R.lo4[d]) * R.g01[i];
     lagrange1d(R.r, nodes, m, v, nullptr);
     // |l| <= 1 inside the box (GLL nodes); outside it the cell is flagged
-    for (int i = 0; i < n1; ++i) wts[task * 12 + i] = fx_from_double(fmin(fmax(v[i], -1.0), 1.0), 0);
+    for (int i = 0; i < n1; ++i) wts[task * 12 + i] = fx_from_double<FX_THETA>(fmin(fmax(v[i], -1.0), 1.0), 0);
     return;
   }
   if (task >= n4 + 9LL * P.ncells) return;
@@ -220,18 +220,22 @@ __global__ void __launch_bounds__(128) cell_prep_kernel(CellParams P, const Thet
 // coefficients t, the (g3, g4) planes of the sample grid are divided among
 // the warps of each group (the groups read the same samples close together,
 // from L1), and the partial sums are added in warp order.  The sums run in
-// 56-bit fixed point on the integer pipe: the samples are scaled per t to
-// |A_t| <= 1/4 and the 1D weights satisfy |l| <= 1 (Lagrange polynomials on GLL
-// nodes) with 1-norms below 2.22 (Lebesgue constants, r <= 10), so the sums
-// over a plane stay below 1.24 and those over the planes below 6.1, inside
-// the bounds of fx56.cuh.  Results are within 2^-54 max |A_t|, the rounding of
-// an FP64 sum, in every form of the assembly.  Bound: the integer
+// 59-bit fixed point on the integer pipe: the samples are scaled per t to
+// |A_t| <= 1/2 and the 1D weights satisfy |l| <= 1 (Lagrange polynomials on GLL
+// nodes) with 1-norms of at most 1.98 (Lebesgue constants, r <= 7), so the sums
+// over a plane stay below 1.95 (their high digit below 2^31) and those over the
+// planes below 7.6 of the 8 that hi hi holds; for r = 8..10 (2.19) the samples
+// take half of that.  The cross sums of r = 6 stay below 49 2^57 + 3.6 2^58 <
+// 2^62.9, those of a warp's planes below 2^62.6; the general form carries
+// after each line.  Bound: the integer
 // multiply-adds.  Measured, the whole phase with the edge functionals, FP64
 // form: 16 cells, n_r = 20: 1.30 -> 0.13 ms (one warp walked the grid
 // alone); 4,096 cells, n_r = 40: 2.60 -> 0.76; 17,424 cells, n_r = 60: 7.7 ->
 // 3.0 (this kernel 1.9; a double-float form on the FP32 pipe took as long
-// and kept 48 bits).  Error against extended precision over max |A_t|: rms
-// 1.2e-16 to 1.6e-16, the FP64 sums' 1.6e-16 to 3.0e-16.
+// and kept 48 bits).  Error against extended precision over max |A_t|, trained
+// models of p = 3 to 8: rms 0.15 to 0.97 of the FP64 sums' (1e-16 to 3.4e-16);
+// with 56 bits and samples of 1/4 it was up to 1.3 of theirs (p = 7, 8), and
+// coefficients far below their largest sample lost up to 12 times as much.
 #define TH_WARPS 7   // r = 6: 49 planes
 __device__ inline float tf32_round_dev(float f) {
   uint32_t u = __float_as_uint(f);
@@ -242,7 +246,7 @@ __device__ inline float tf32_round_dev(float f) {
 __device__ __forceinline__ int2 fx_mul(int2 a, int2 b) {   // |a|, |b| <= 1
   long long hh = 0, x = 0;
   fx_mad(hh, x, a, b);
-  return fx_digits(fx_sum(hh, x));
+  return fx_digits<FX_THETA>(fx_sum<FX_THETA>(hh, x));
 }
 
 // NS = ceil(n_r / 32) lane slots per coefficient; N1 = r + 1 when known at
@@ -322,13 +326,21 @@ __global__ void __launch_bounds__(32 * TH_WARPS * CG) theta_kernel(
             for (int j = 0; j < CT; ++j) fx_mad(ih[s][j], ix[s][j], a, wc[j * n2 + g2 * n1 + g1]);
           }
         }
+#pragma unroll
+        for (int s = 0; s < NS; ++s)   // carry: 64 terms and more could pass 2^63
+#pragma unroll
+          for (int j = 0; j < CT; ++j) {
+            ih[s][j] += ix[s][j] >> (FX_THETA - 30);
+            ix[s][j] &= (1LL << (FX_THETA - 30)) - 1;
+          }
       }
     }
 #pragma unroll
     for (int j = 0; j < CT; ++j) {
       const int2 w = w34[(cg * CT + j) * n2 + g34];
 #pragma unroll
-      for (int s = 0; s < NS; ++s) fx_mad(oh[s][j], ox[s][j], fx_digits(fx_sum(ih[s][j], ix[s][j])), w);
+      for (int s = 0; s < NS; ++s) 
+        fx_mad(oh[s][j], ox[s][j], fx_digits<FX_THETA>(fx_sum<FX_THETA>(ih[s][j], ix[s][j])), w);
     }
   }
   __syncthreads();   // the weights are read no more: their memory takes the partial sums
@@ -336,7 +348,8 @@ __global__ void __launch_bounds__(32 * TH_WARPS * CG) theta_kernel(
   for (int s = 0; s < NS; ++s)
 #pragma unroll
     for (int j = 0; j < CT; ++j)
-      part[(warp * NC + cg * CT + j) * (32 * NS) + lane + 32 * s] = fx_sum(oh[s][j], ox[s][j]);
+      part[(warp * NC + cg * CT + j) * (32 * NS) + lane + 32 * s] =
+          fx_sum<FX_THETA>(oh[s][j], ox[s][j]);
   __syncthreads();
   for (int i = tid; i < NC * 128; i += nt) {
     const int j = i >> 7, t = i & 127;   // slot t of theta: 0 rho, 1.. the coefficients
@@ -350,7 +363,7 @@ __global__ void __launch_bounds__(32 * TH_WARPS * CG) theta_kernel(
 #pragma unroll
       for (int w = 0; w < TH_WARPS; ++w) sum += part[(w * NC + j) * (32 * NS) + t - 1];
       const int e = R.at_exp[t - 1];
-      v = (1.0 - P.rho) * (e == FX_NAN ? nan("") : ldexp((double)sum, e - FX_BITS));
+      v = (1.0 - P.rho) * (e == FX_NAN ? nan("") : ldexp((double)sum, e - FX_THETA));
     }
     if (t <= nr) theta[128 * c + t] = v;
     // TF32 hi / lo split of the tensor-core slots of theta (0 and 2..; slot 1

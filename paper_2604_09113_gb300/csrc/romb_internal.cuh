@@ -52,7 +52,7 @@ struct RombRom {
   int kpad16 = 0;              // n_r+1 rounded up to the BF16 MMA K step (16)
   double* A = nullptr;         // [n_r][(r+1)^4]
   double* At = nullptr;        // [(r+1)^4][n_r]
-  int* rexp = nullptr;         // [n_r+1] exponents of the rows of U' (FX_NAN: not finite)
+  int* rexp = nullptr;         // [n_r+1] scales of the rows of U' in the FP64 form (exponents; FX_NAN: not finite)
   int2* Atfx = nullptr;        // [(r+1)^4][n_r] A transposed, fixed point (fx56.cuh) scaled by 2^-at_exp[t]
   int* at_exp = nullptr;       // [n_r]
   int kpad = 0;                // n_r+1 rounded up for the tensor-core K dimension

@@ -57,7 +57,7 @@ struct RombRom {
   int* at_exp = nullptr;       // [n_r]
   int kpad = 0;                // n_r+1 rounded up for the tensor-core K dimension
   unsigned char* Udig = nullptr;   // U' as BF16 digits of the FP64 form, and the exponents of its
-  int* pexp = nullptr;             // pairs (assemble_digits.cu; built on the first FP64 assembly)
+  int* pexp = nullptr;             // pairs (built by the first FP64 assembly, given back when memory is short)
   // reduced model of the force integrals J(mu) (file version 2; absent: null)
   int force_nf = 0, force_rf = 0;
   double* force_U = nullptr;   // [r_f][n_f], n_f = 4 (p+1) (q+1): J[e][s][k]
@@ -267,7 +267,9 @@ struct romb_ctx {
 // allocation helpers (respect the budget)
 romb_status romb_alloc(romb_ctx* c, void** p, size_t bytes);
 romb_status romb_alloc_persist(romb_ctx* c, void** p, size_t bytes);
-void romb_free_persist(romb_ctx* c, void* p);
+romb_status romb_alloc_optional(romb_ctx* c, void** p, size_t bytes);   // the digit tiles
+void romb_free_digits(romb_ctx* c, RombRom& R);
+bool romb_release_digits(romb_ctx* c, bool all);
 void romb_free_lattice(romb_ctx* c);
 template <class T>
 inline romb_status romb_alloc_t(romb_ctx* c, T** p, size_t n) {

@@ -260,9 +260,9 @@ romb_status romb_set_precond_precision(romb_ctx* ctx, int mode);
  * agree to rounding; what they differ by shows where a result cancels: the
  * interior displacements of nearly void cells follow the last bits of K (its
  * row sums against rho), and dc/dctrl of romb_compliance_grad carries that at
- * ~1e-9 on a 64 x 64 lattice.  Runs that are compared with stored gradients
- * choose 1 (the torch binding of the compliance does).  The choice stays
- * with the context.  Errors: ROMB_E_ARG. */
+ * ~1e-9 on a 64 x 64 lattice, as far as either is from a 64-bit evaluation.
+ * Runs that are compared bit by bit with gradients stored by the FP64 pipe
+ * choose 1.  The choice stays with the context.  Errors: ROMB_E_ARG. */
 romb_status romb_set_fp64_arithmetic(romb_ctx* ctx, int on);
 
 /* A constant body force (bx, by) per unit physical area on the solid part of

@@ -9,6 +9,11 @@ romb_bddc_solve and romb_compliance_grad of libromb on the caller's context;
 the backward pass scales the gradient that call returned.  Inputs on a CUDA
 device are passed to the library in place (device memory kind), CPU tensors
 as host arrays; gradients come back on the inputs' device in float64.
+
+The arithmetic is the context's (romb_set_fp64_arithmetic) and stays so.  dc/dctrl
+of a large lattice carries the last bits of K: between the default and the FP64
+pipe it moves by 1e-9 on 64 x 64 cells and by 3e-11 to 1.3e-10 on 1,200 to 2,500,
+as far as either is from a 64-bit evaluation (dc/dmu 1e-10 and 1e-11).
 """
 from __future__ import annotations
 
@@ -17,8 +22,7 @@ import types
 import numpy as np
 import torch
 
-from . import (ROMB_FP64, romb_assemble, romb_bddc_solve, romb_compliance_grad, romb_factor,
-               romb_set_fp64_arithmetic)
+from . import (ROMB_FP64, romb_assemble, romb_bddc_solve, romb_compliance_grad, romb_factor)
 
 
 class Compliance(torch.autograd.Function):
@@ -49,10 +53,6 @@ class Compliance(torch.autograd.Function):
             darr = None
             view.ctrl, view.mu = ctrl_d.numpy(), mu_d.numpy()
             out = None
-        # dc/dctrl on a large lattice carries the last bits of K at ~1e-9: they
-        # stay those of the FP64 pipe, so that gradients match stored ones and
-        # further solves of this context match the gradient's
-        romb_set_fp64_arithmetic(session.h, True)
         romb_assemble(session.h, view, precision, device_arrays=darr)
         romb_factor(session.h)
         romb_bddc_solve(session.h, nodes, rtol=rtol, maxit=maxit, out=out)

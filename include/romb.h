@@ -146,7 +146,8 @@ romb_status romb_assemble(romb_ctx* ctx, const romb_lattice* lat, romb_precision
 /* As romb_assemble, but with caller-supplied dense cell matrices
  * K[ncells][ndof][ndof] (ndof = 2 (p+1)^2, local DoF 2k+i; ncells = nx*ny,
  * or the present cells in increasing grid index), e.g. from full trimmed
- * quadrature (the unaccelerated baseline of Sec. 5.1). */
+ * quadrature (the unaccelerated baseline of Sec. 5.1).  They are taken as they
+ * are; romb_set_fp64_arithmetic chooses the arithmetic of their factorisation. */
 romb_status romb_assemble_host_K(romb_ctx* ctx, const romb_lattice* lat, const double* K);
 
 /* BDDC set-up (Sec. 3): per cell the Cholesky factor of K_II and the Schur
@@ -252,11 +253,13 @@ romb_status romb_set_load_form(romb_ctx* ctx, int form);
 enum { ROMB_PRECOND_AUTO = -1, ROMB_PRECOND_FP64 = 0, ROMB_PRECOND_FP32 = 1 };
 romb_status romb_set_precond_precision(romb_ctx* ctx, int mode);
 
-/* The arithmetic of the FP64 form from the next romb_assemble on.  0 (default):
- * theta in 59-bit fixed point, the contraction by exact digit products on the
- * tensor cores, and the matrix products of romb_factor in 56-bit integers, each
- * within the rounding of the FP64 sums.  1: all on the FP64 pipe, every sum in
- * one fixed order (the assembly at ~10 times the time).  The two
+/* The FP64 arithmetic from the next romb_assemble or romb_assemble_host_K on:
+ * of theta and K in the form ROMB_FP64, and of romb_factor after every form and
+ * with the caller's own matrices.  0 (default): theta in 59-bit fixed point, the
+ * contraction by exact digit products on the tensor cores, and the matrix
+ * products of romb_factor in 56-bit integers, each within the rounding of the
+ * FP64 sums.  1: all on the FP64 pipe, every sum in one fixed order (the
+ * assembly at ~10 times the time).  The two
  * agree to rounding; what they differ by shows where a result cancels: the
  * interior displacements of nearly void cells follow the last bits of K (its
  * row sums against rho), and dc/dctrl of romb_compliance_grad carries that at

@@ -214,9 +214,10 @@ def romb_set_exact_fallback(ctx, max_cells: int) -> None:
 
 
 def romb_set_fp64_arithmetic(ctx, on: bool) -> None:
-    """The FP64 form's theta and contraction on the FP64 pipe in one fixed order
-    (True), or in fixed point and digit products (False, the default; faster,
-    equal to rounding): from the next romb_assemble on."""
+    """The FP64 form's theta and contraction, and romb_factor of every form and of
+    the caller's matrices, on the FP64 pipe in one fixed order (True), or in
+    fixed point and digit products (False, the default; faster, equal to
+    rounding): from the next romb_assemble or romb_assemble_host_K on."""
     _check(_lib.romb_set_fp64_arithmetic(ctx, int(on)), "romb_set_fp64_arithmetic")
 
 

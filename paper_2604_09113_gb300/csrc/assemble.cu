@@ -553,7 +553,7 @@ romb_status launch_theta(romb_ctx* c) {
       P, d_fams, c->d_slot, c->d_ctrl, c->d_mu, c->d_wts, c->d_chat, c->d_chat32, c->d_flags);
   ++c->launches;
   ROMB_CUDA(cudaGetLastError());
-  if (c->plain64) return launch_theta_fp64(c);
+  if (c->plain64 && c->prec == ROMB_FP64) return launch_theta_fp64(c);
   // one launch per group of models that share the kernel's template arguments
   bool done[ROMB_MAX_MODELS] = {false};
   for (int f0 = 0; f0 < ROMB_MAX_MODELS; ++f0) {

@@ -240,7 +240,7 @@ struct romb_ctx {
   bool pre32 = false;
   int precond_mode = -1;        // romb_set_precond_precision (survives a new lattice)
   bool fp64_pipe = false;       // romb_set_fp64_arithmetic (survives a new lattice)
-  bool plain64 = false;         // the cell matrices were assembled that way
+  bool plain64 = false;         // the choice at the last assembly: of the FP64 form's theta and K, and of romb_factor
   int fallback_max = 64;        // romb_set_exact_fallback (survives a new lattice)
   // exact tensors of the fallback, row 1 of U' in the half layout, keyed by
   // (family, basis, p, q, mu): a cell met again skips the quadrature

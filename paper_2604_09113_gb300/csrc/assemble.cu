@@ -249,12 +249,17 @@ __device__ __forceinline__ int2 fx_mul(int2 a, int2 b) {   // |a|, |b| <= 1
   return fx_digits<FX_THETA>(fx_sum<FX_THETA>(hh, x));
 }
 
+// the models of one launch: slot[k] owns CTAs from cta[k] to cta[k + 1]
+struct ThetaCtas {
+  int slot[ROMB_MAX_MODELS], cta[ROMB_MAX_MODELS + 1];
+};
+
 // NS = ceil(n_r / 32) lane slots per coefficient; N1 = r + 1 when known at
 // compile time (0: from the model), so that the loads of a line (g2, g3, g4)
 // are issued together.
 template <int NS, int CT, int CG, int N1>
 __global__ void __launch_bounds__(32 * TH_WARPS * CG) theta_kernel(
-    CellParams P, const ThetaFams* __restrict__ Fams, const int* __restrict__ models,
+    CellParams P, const ThetaFams* __restrict__ Fams, const __grid_constant__ ThetaCtas models,
     const int2* __restrict__ wts, double* __restrict__ theta, float* __restrict__ th_hi,
     float* __restrict__ th_lo) {
   constexpr int NC = CT * CG;
@@ -264,14 +269,13 @@ __global__ void __launch_bounds__(32 * TH_WARPS * CG) theta_kernel(
   long long* part = reinterpret_cast<long long*>(th_smem);   // [TH_WARPS][NC][32 NS]
   const int tid = threadIdx.x, lane = tid & 31, warp = (tid >> 5) % TH_WARPS, cg = (tid >> 5) / TH_WARPS;
   const int nt = blockDim.x;
-  // the model of this CTA: models[2 k] owns CTAs from models[2 k + 1] on
-  int k = 0;
-  while ((int)blockIdx.x >= models[2 * k + 3]) ++k;
-  const int fi = models[2 * k];
+  int k = 0;   // the model of this CTA
+  while ((int)blockIdx.x >= models.cta[k + 1]) ++k;
+  const int fi = models.slot[k];
   const RomDev& R = Fams->rom[fi];
   const int* __restrict__ list = Fams->list[fi];
   const int count = Fams->count[fi];
-  const int first = ((int)blockIdx.x - models[2 * k + 1]) * NC;
+  const int first = ((int)blockIdx.x - models.cta[k]) * NC;
   const int n1 = N1 > 0 ? N1 : R.r + 1, nr = R.n_r;
   for (int i = tid; i < NC * 48; i += nt) {
     const int j = i / 48;
@@ -547,7 +551,8 @@ romb_status launch_theta(romb_ctx* c) {
     F.count[f] = counts[f];
   }
   ThetaFams* d_fams = reinterpret_cast<ThetaFams*>(c->d_fams);
-  // pageable source: staged before the call returns
+  // the table of the context: the copy is done before the next call writes it
+  // again (the wait for the counts above)
   ROMB_CUDA(cudaMemcpyAsync(d_fams, &F, sizeof(F), cudaMemcpyHostToDevice, c->stream));
   cell_prep_kernel<<<(int)((13LL * c->ncells + 127) / 128), 128, 0, c->stream>>>(
       P, d_fams, c->d_slot, c->d_ctrl, c->d_mu, c->d_wts, c->d_chat, c->d_chat32, c->d_flags);
@@ -566,28 +571,25 @@ romb_status launch_theta(romb_ctx* c) {
     // CTAs spread over the SMs.
     const bool few = c->ncells < 8 * c->sms;
     const int ct = few || ns > 2 ? 2 : 4, cg = few ? 1 : 2, nc = ct * cg;
-    std::vector<int> models;   // (slot, first CTA) pairs, then (-1, CTAs)
-    int grid = 0, n1max = 0;
+    ThetaCtas models;
+    int grid = 0, n1max = 0, nm = 0;
     for (int f = f0; f < ROMB_MAX_MODELS; ++f) {
       const RombRom& Rr = c->roms[f];
       if (done[f] || counts[f] == 0 || (Rr.n_r + 31) / 32 != ns || (Rr.r == 6) != r6) continue;
       done[f] = true;
-      models.push_back(f);
-      models.push_back(grid);
+      models.slot[nm] = f;
+      models.cta[nm++] = grid;
       n1max = std::max(n1max, Rr.r + 1);
       grid += (counts[f] + nc - 1) / nc;
     }
-    models.push_back(-1);
-    models.push_back(grid);
-    int* d_models = reinterpret_cast<int*>(d_fams + 1);   // rewritten in stream order
-    ROMB_CUDA(cudaMemcpyAsync(d_models, models.data(), 4 * models.size(), cudaMemcpyHostToDevice, c->stream));
+    models.cta[nm] = grid;
 #define TH_(NS_) (few ? (r6 ? theta_kernel<NS_, 2, 1, 7> : theta_kernel<NS_, 2, 1, 0>) \
                       : (r6 ? theta_kernel<NS_, NS_ <= 2 ? 4 : 2, 2, 7> : theta_kernel<NS_, NS_ <= 2 ? 4 : 2, 2, 0>))
     auto k = ns <= 1 ? TH_(1) : ns == 2 ? TH_(2) : ns == 3 ? TH_(3) : TH_(4);
 #undef TH_
     const size_t smem = 8 * std::max((size_t)2 * nc * n1max * n1max, (size_t)TH_WARPS * nc * 32 * ns);
     ROMB_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    k<<<grid, 32 * TH_WARPS * cg, smem, c->stream>>>(P, d_fams, d_models, c->d_wts, c->d_theta, c->d_theta_hi,
+    k<<<grid, 32 * TH_WARPS * cg, smem, c->stream>>>(P, d_fams, models, c->d_wts, c->d_theta, c->d_theta_hi,
                                                      c->d_theta_lo);
     ++c->launches;
     ROMB_CUDA(cudaGetLastError());
@@ -595,8 +597,8 @@ romb_status launch_theta(romb_ctx* c) {
   return ROMB_OK;
 }
 
-// bytes of the device table of launch_theta: the models, then one launch's CTA list
-size_t theta_table_bytes() { return sizeof(ThetaFams) + 8 * (ROMB_MAX_MODELS + 1); }
+// bytes of the device table of launch_theta
+size_t theta_table_bytes() { return sizeof(ThetaFams); }
 
 romb_status launch_assemble_fp64(romb_ctx* c) {
   if (!c->plain64) {

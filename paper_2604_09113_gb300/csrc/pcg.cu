@@ -1025,8 +1025,11 @@ romb_status pcg_begin(romb_ctx* c, PcgLane& L, const double* tr, bool tr_on_devi
     QNodes QN;
     memset(&QN, 0, sizeof(QN));
     gll_nodes01(c->q, QN.n);
-    std::vector<ForceRomDev> tab(ROMB_MAX_MODELS);
-    memset(tab.data(), 0, sizeof(ForceRomDev) * tab.size());
+    // kept with the lane: the copy below may still read it when this call has
+    // returned.  The solve waits for the lane before the next one writes it again.
+    L.h_forcetab.resize(sizeof(ForceRomDev) * ROMB_MAX_MODELS);
+    ForceRomDev* tab = reinterpret_cast<ForceRomDev*>(L.h_forcetab.data());
+    memset(tab, 0, L.h_forcetab.size());
     for (int f = 0; f < ROMB_MAX_MODELS; ++f) {
       if (c->famcount[f] == 0) continue;
       const RombRom& R = c->roms[f];
@@ -1051,8 +1054,7 @@ romb_status pcg_begin(romb_ctx* c, PcgLane& L, const double* tr, bool tr_on_devi
       romb_status s = romb_alloc_t(c, &L.d_forcetab, sizeof(ForceRomDev) * ROMB_MAX_MODELS);
       if (s != ROMB_OK) return s;
     }
-    // pageable source: the call returns once the table has been staged
-    ROMB_CUDA(cudaMemcpyAsync(L.d_forcetab, tab.data(), sizeof(ForceRomDev) * ROMB_MAX_MODELS,
+    ROMB_CUDA(cudaMemcpyAsync(L.d_forcetab, tab, sizeof(ForceRomDev) * ROMB_MAX_MODELS,
                               cudaMemcpyHostToDevice, L.stream));
     const long long nedges = 2LL * c->ny + 2LL * c->nx;
     loads_rom_kernel<<<(int)nedges, 32 * FT_WARPS, 0, L.stream>>>(

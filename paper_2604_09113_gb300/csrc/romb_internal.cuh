@@ -133,6 +133,7 @@ struct PcgLane {
   double* d_u = nullptr;           // nodal output [nodes][2]
   double* d_traction = nullptr;    // [4][2]
   unsigned char* d_forcetab = nullptr;   // reduced force models by slot (loads_rom_kernel)
+  std::vector<unsigned char> h_forcetab; // its host copy
   double* d_fI = nullptr;       // [cells][nI] interior body loads, then L^-1 f_I (recovery)
   bool body_on = false;         // this solve carries body forces
   double* nd_ybuf = nullptr;       // coarse-solve update vectors

@@ -264,9 +264,18 @@ romb_status romb_set_precond_precision(romb_ctx* ctx, int mode);
  * interior displacements of nearly void cells follow the last bits of K (its
  * row sums against rho), and dc/dctrl of romb_compliance_grad carries that at
  * ~1e-9 on a 64 x 64 lattice, as far as either is from a 64-bit evaluation.
- * Runs that are compared bit by bit with gradients stored by the FP64 pipe
- * choose 1.  The choice stays with the context.  Errors: ROMB_E_ARG. */
+ * The choice stays with the context, and nothing but this call changes it.
+ * Errors: ROMB_E_ARG. */
 romb_status romb_set_fp64_arithmetic(romb_ctx* ctx, int on);
+
+/* For a gradient that is compared with stored ones: where romb_set_fp64_arithmetic
+ * has never been called, the FP64 form works as after romb_set_fp64_arithmetic(ctx,
+ * 1) from the next romb_assemble on until a lattice of another shape is assembled,
+ * so that the values and gradients of one optimisation are those of one
+ * arithmetic.  A choice made by romb_set_fp64_arithmetic, 0 or 1, comes first,
+ * before this call and after it.  The torch binding of the compliance calls it
+ * for ROMB_FP64.  Errors: ROMB_E_ARG for a null context. */
+romb_status romb_gradient_arithmetic(romb_ctx* ctx);
 
 /* A constant body force (bx, by) per unit physical area on the solid part of
  * every cell (the volume term of Eq. SPEED L ext): with b_hat = det J b at the

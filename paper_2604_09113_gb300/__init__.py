@@ -76,6 +76,7 @@ def _load():
         "romb_set_precond_precision": ([P, I], I),
         "romb_set_exact_fallback": ([P, I], I),
         "romb_set_fp64_arithmetic": ([P, I], I),
+        "romb_gradient_arithmetic": ([P], I),
         "romb_train_gpu_clustered": ([I, ctypes.POINTER(RombTrainSpec), I, P, I, ctypes.c_char_p], I),
     }
     for name, (args, res) in sig.items():
@@ -219,6 +220,12 @@ def romb_set_fp64_arithmetic(ctx, on: bool) -> None:
     fixed point and digit products (False, the default; faster, equal to
     rounding): from the next romb_assemble or romb_assemble_host_K on."""
     _check(_lib.romb_set_fp64_arithmetic(ctx, int(on)), "romb_set_fp64_arithmetic")
+
+
+def romb_gradient_arithmetic(ctx) -> None:
+    """Where romb_set_fp64_arithmetic has never been called: the FP64 form on the
+    FP64 pipe from the next romb_assemble on, for lattices of that shape."""
+    _check(_lib.romb_gradient_arithmetic(ctx), "romb_gradient_arithmetic")
 
 
 def romb_set_body_force(ctx, bx: float, by: float) -> None:

@@ -10,10 +10,12 @@ the backward pass scales the gradient that call returned.  Inputs on a CUDA
 device are passed to the library in place (device memory kind), CPU tensors
 as host arrays; gradients come back on the inputs' device in float64.
 
-The arithmetic is the context's (romb_set_fp64_arithmetic) and stays so.  dc/dctrl
-of a large lattice carries the last bits of K: between the default and the FP64
-pipe it moves by 1e-9 on 64 x 64 cells and by 3e-11 to 1.3e-10 on 1,200 to 2,500,
-as far as either is from a 64-bit evaluation (dc/dmu 1e-10 and 1e-11).
+dc/dctrl of a large lattice carries the last bits of K: between the default FP64
+arithmetic and the FP64 pipe it moves by 1e-9 on 64 x 64 cells, as far as either is
+from a 64-bit evaluation.  Gradients and the FP64 steps that follow on the same
+lattice are therefore those of the FP64 pipe, as stored ones are
+(romb_gradient_arithmetic); a choice made by romb_set_fp64_arithmetic comes first:
+romb_set_fp64_arithmetic(session.h, False), once, gives both in the default.
 """
 from __future__ import annotations
 
@@ -22,7 +24,8 @@ import types
 import numpy as np
 import torch
 
-from . import (ROMB_FP64, romb_assemble, romb_bddc_solve, romb_compliance_grad, romb_factor)
+from . import (ROMB_FP64, romb_assemble, romb_bddc_solve, romb_compliance_grad, romb_factor,
+               romb_gradient_arithmetic)
 
 
 class Compliance(torch.autograd.Function):
@@ -53,6 +56,8 @@ class Compliance(torch.autograd.Function):
             darr = None
             view.ctrl, view.mu = ctrl_d.numpy(), mu_d.numpy()
             out = None
+        if precision == ROMB_FP64:
+            romb_gradient_arithmetic(session.h)
         romb_assemble(session.h, view, precision, device_arrays=darr)
         romb_factor(session.h)
         romb_bddc_solve(session.h, nodes, rtol=rtol, maxit=maxit, out=out)

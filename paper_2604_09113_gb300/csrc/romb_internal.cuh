@@ -240,7 +240,9 @@ struct romb_ctx {
   // the coarse solve's B) in FP32, set by romb_factor
   bool pre32 = false;
   int precond_mode = -1;        // romb_set_precond_precision (survives a new lattice)
-  bool fp64_pipe = false;       // romb_set_fp64_arithmetic (survives a new lattice)
+  int fp64_choice = -1;         // romb_set_fp64_arithmetic: 0, 1, -1 never called (survives a new lattice)
+  bool gradient_next = false;   // romb_gradient_arithmetic, taken up by the next romb_assemble
+  bool gradient_pipe = false;   // and kept until the lattice's shape changes
   bool plain64 = false;         // the choice at the last assembly: of the FP64 form's theta and K, and of romb_factor
   int fallback_max = 64;        // romb_set_exact_fallback (survives a new lattice)
   // exact tensors of the fallback, row 1 of U' in the half layout, keyed by

@@ -42,6 +42,31 @@ def test_a_gradient_leaves_the_choice(pipe, precision):
         assert np.array_equal(_k(ctx, lat), before)
 
 
+@pytest.mark.parametrize("precision", ["ROMB_FP64", "ROMB_FP32_SPLIT"])
+def test_without_a_choice_a_gradient_holds_for_its_lattice(precision):
+    """Where nobody chose, a gradient in the FP64 form takes the FP64 pipe for the
+    lattices of its shape; another shape, and a split form, leave the default.  A
+    choice made afterwards holds."""
+    lat, other = _lat(4), _lat(4, 3, 3)
+    _, path = small_rom(0, 4, 0.18, 0.40, 20, 12, 1)
+    with romb.Context(0) as ctx:
+        romb.romb_train_load(ctx.h, path)
+        default, default_other = _k(ctx, lat), _k(ctx, other)
+        ctrl = torch.tensor(lat.ctrl, requires_grad=True)
+        mu = torch.tensor(lat.mu, requires_grad=True)
+        compliance(ctx, lat, ctrl, mu, getattr(romb, precision), rtol=1e-8).backward()
+        assert np.array_equal(_k(ctx, lat), default) == (precision != "ROMB_FP64")
+        assert np.array_equal(_k(ctx, other), default_other)
+        bad = _lat(4, 3, 3)
+        bad.rho = -1.0
+        with pytest.raises(romb.RombError):   # a refused gradient leaves nothing behind
+            compliance(ctx, bad, torch.tensor(bad.ctrl), torch.tensor(bad.mu), getattr(romb, precision), rtol=1e-8)
+        assert np.array_equal(_k(ctx, lat), default)
+        compliance(ctx, lat, ctrl, mu, getattr(romb, precision), rtol=1e-8).backward()
+        romb.romb_set_fp64_arithmetic(ctx.h, False)
+        assert np.array_equal(_k(ctx, lat), default)
+
+
 @pytest.mark.parametrize("source", ["given", "ROMB_FP32_SPLIT", "ROMB_BF16_SPLIT"])
 def test_choice_reaches_every_factorisation(source):
     """The factorisation of the caller's own matrices and of the split forms

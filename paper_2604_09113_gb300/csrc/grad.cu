@@ -73,7 +73,7 @@ __global__ void __launch_bounds__(256) theta_fp64_kernel(CellParams P, const dou
 // cells take fewer cells per CTA, so that the sequence of pairs is walked on
 // all SMs.  Bound: FP64 issue (2 K 36 + 600 FMA per cell and pair).  Before, 36
 // of 64 lanes worked, in CTAs one to an SM: 4,096 cells, n_r = 40: 61.5 -> 36.8 ms
-// (29 ms of FP64 issue); 35 cells: 9.3 -> 7.2.
+// (17.8 G FMA: 34 ms at the measured FP64 rate); 35 cells: 9.3 -> 7.2.
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
 }

@@ -21,7 +21,7 @@ def _lattices(p):
     return out
 
 
-def _work(budget, pipe, paths, lats):
+def _steps(budget, pipe, paths, lats):
     """Two lattices, the second larger: assembled, factorised and solved with two
     load sets twice, then a gradient."""
     out = []
@@ -44,7 +44,7 @@ def _work(budget, pipe, paths, lats):
 
 def _fits(budget, *args):
     try:
-        _work(budget, *args)
+        _steps(budget, *args)
     except romb.RombError as e:
         assert "memory" in str(e), e
         return False
@@ -55,7 +55,7 @@ def test_tiles_leave_every_budget_as_it_was():
     p = 4
     paths = [small_rom(f, p, 0.18, 0.40, 20, 12, 1)[1] for f in (0, 1)]
     lats = _lattices(p)
-    ref = _work(0, False, paths, lats)
+    ref = _steps(0, False, paths, lats)
     lo, hi = 1 << 16, 1 << 28   # the least budget of the work without tiles, to 4 KB
     assert _fits(hi, True, paths, lats) and not _fits(lo, True, paths, lats)
     while hi - lo > 4096:
@@ -63,6 +63,6 @@ def test_tiles_leave_every_budget_as_it_was():
         lo, hi = (lo, mid) if _fits(mid, True, paths, lats) else (mid, hi)
     tiles = 325 * 8 * 40 * 2 * 16   # of one model: pairs, digits, rows, bytes, K padded
     for extra in (0, tiles // 2, tiles + tiles // 2, 2 * tiles + 65536):
-        got = _work(hi + extra, False, paths, lats)
+        got = _steps(hi + extra, False, paths, lats)
         for a, b in zip(got, ref):
             assert np.abs(a - b).max() <= 1e-8 * np.abs(b).max(), extra
